@@ -830,12 +830,10 @@ def roofline_of(st, ms_total, precision, wl, fp64_peak=None):
         nm = int(os.environ.get("QSI_MIXED_MODULI", MODULI["mixed"])) if precision == "mixed" else 17
         sweep = min(prod_flops, st["tc_flops"])
         newton = st["tc_flops"] - sweep
-        # of an inversion's six Newton products one takes 17 moduli, the corrections 13
-        newton_moduli = (17.0 + 5 * 13.0) / 6.0
         if precision == "split3":
-            bf16_work = 6.0 * sweep + newton_moduli * newton
+            bf16_work = 6.0 * sweep + 17.0 * newton
         else:
-            bf16_work = nm * sweep + newton_moduli * newton
+            bf16_work = nm * sweep + 17.0 * newton
         cands.append(dict(kernel="tc_mma_kernel", what="tcgen05 BF16 products of the FP64-emulated block products",
                           ms=st["tc_ms"], launches=st["tc_launches"], flops=sweep, bound="tensor",
                           peak=bf16, peak_source="of measured: bf16_tflops_sustained in MEASURED_PEAKS.json",
