@@ -85,3 +85,26 @@ def test_small_inverse_reports_the_singular_column(ctx, b, col):
         ctx.synchronize()
     assert e.value.status == qsi.ERR_SINGULAR
     f.close()
+
+
+@pytest.mark.parametrize("b,points", [(5, 97), (32, 97), (33, 65), (64, 65)])
+def test_wide_batches_of_small_blocks_give_the_bits_of_narrow_ones(ctx, b, points):
+    """One CTA per block above 96 (b <= 32) or 64 blocks, a cluster per block up to
+    there: a batch on either side of the line, the same bits."""
+    import torch
+    from paper_2601_04904_gb300 import inputs, qsi
+
+    n = 2
+    Hd = qsi.to_device(inputs.hamiltonian(n, b, 0))
+    E, g = inputs.energy_grid(points)
+    B = qsi.batched_zeros(points, n, b, 0)
+    B["diag"].copy_(torch.eye(b, dtype=torch.complex128, device="cuda") * 1j)
+    torch.cuda.synchronize()
+    wide = ctx.selquad_batched(Hd, E, 1e-3, g, B, precision=qsi.FP64)
+    half = points // 2 + 1
+    narrow = [ctx.selquad_batched(Hd, E[s], 1e-3, g[s], {k: v[s].contiguous() for k, v in B.items()},
+                                  precision=qsi.FP64) for s in (slice(0, half), slice(half, points))]
+    ctx.synchronize()
+    for i in (0, 1):
+        for key in qsi.KEYS:
+            assert (torch.cat([narrow[0][i][key], narrow[1][i][key]]) == wide[i][key]).all(), key
