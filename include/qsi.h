@@ -28,7 +28,7 @@
  * Errors: every call returns a qsi_status and never aborts or throws across
  * the ABI.  Work is asynchronous on the context's stream; errors found on the
  * device (a zero or non-finite pivot in a diagonal-block or tip inversion; a
- * tensor-core kernel whose bounded internal wait ran out) are reported by the
+ * kernel whose bounded internal wait ran out) are reported by the
  * next qsi_synchronize() (or by the *_host call, which synchronises) as
  * QSI_ERR_SINGULAR (block index in qsi_last_error()) or QSI_ERR_TIMEOUT.
  * After QSI_ERR_SINGULAR the outputs hold non-finite values but the context
@@ -440,7 +440,10 @@ qsi_status qsi_set_flags(qsi_ctx *ctx, uint32_t flags);
  * and the context stays usable.  This call queues one kernel on ctx's stream
  * that performs such a wait, with limit_us microseconds (1..2e6), on an
  * mbarrier that nothing arrives at, so that the path can be exercised without
- * a fault.  Returns QSI_OK once queued (QSI_ERR_ARG for a bad limit). */
+ * a fault.  Returns QSI_OK once queued (QSI_ERR_ARG for a bad limit).
+ * The waits of the inversion kernels between the CTAs of a cluster take their
+ * limit, 2 s, from QSI_INV_WAIT_NS in the environment where that is set (0: no
+ * wait waits).  A timeout is reported before any other error of the same work. */
 qsi_status qsi_selftest_wait_timeout(qsi_ctx *ctx, int32_t limit_us);
 
 /* Largest block size accepted by qsi_block_inverse_noalloc. */

@@ -555,8 +555,10 @@ qsi_status qsi_synchronize(qsi_ctx *ctx) {
   CK(cudaMemcpy(&h, ctx->d_status, sizeof h, cudaMemcpyDeviceToHost));
   if (h.code != 0 || h.tc_err != 0) {
     CK(cudaMemset(ctx->d_status, 0, sizeof h));
-    if (h.code == 0 && h.tc_err != 0)
-      return fail(ctx, QSI_ERR_TIMEOUT, "tensor-core kernel: bounded wait ran out (stage %d)", h.tc_err);
+    // first: whatever else was recorded may come from what the wait was to bring
+    if (h.tc_err != 0)
+      return fail(ctx, QSI_ERR_TIMEOUT, "%s: bounded wait ran out (stage %d)",
+                  h.tc_err == QSI_STAGE_GJ32 ? "FP32 Gauss-Jordan" : "tensor-core kernel", h.tc_err);
     if (h.code == QSI_ERR_SINGULAR)
       return fail(ctx, QSI_ERR_SINGULAR, "singular pivot: block %d (tip if %s), column %d", h.tag, "tag == n_blocks",
                   h.info);

@@ -16,8 +16,17 @@ struct QsiDevStatus {
   int code;
   int tag;
   int info;
-  int tc_err;  // tensor-core kernel: a bounded wait ran out (QSI_ERR_TIMEOUT)
+  int tc_err;  // a bounded wait ran out (QSI_ERR_TIMEOUT), in which stage
 };
+// stages 1..5: the tensor-core products
+constexpr int QSI_STAGE_GJ32 = 6;        // cluster form of the FP32 Gauss-Jordan
+
+// Limit of a wait inside the inversion kernels, 2 s; QSI_INV_WAIT_NS in the
+// environment sets another one (0: no wait waits, all count as run out), for tests.
+inline unsigned long long qsi_inv_wait_ns() {
+  const char *v = getenv("QSI_INV_WAIT_NS");
+  return v ? strtoull(v, nullptr, 10) : 2000000000ull;
+}
 
 // ---------------------------------------------------------------------------
 // Grouped complex GEMM: for every problem p of a group and every batch index z
