@@ -460,7 +460,8 @@ qsi_status qsi_selftest_wait_timeout(qsi_ctx *ctx, int32_t limit_us);
  * A, Ainv: device pointers to b x b row-major complex128 (16-byte aligned);
  * they may be the same pointer (in-place).  info: device pointer to one
  * int32 that receives 0, or 1 + the first pivot column that was zero or
- * non-finite (Ainv then holds non-finite values).  Work is queued on
+ * non-finite (Ainv then holds non-finite values), or -1 if a bounded wait
+ * inside the kernel ran out (Ainv is then no inverse).  Work is queued on
  * cuda_stream (a cudaStream_t; NULL = legacy default stream) for the current
  * device.  The first call on each device looks up the scratch array's device
  * address (cudaGetSymbolAddress) and caches it: make that first call before

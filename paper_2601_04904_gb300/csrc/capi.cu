@@ -558,7 +558,10 @@ qsi_status qsi_synchronize(qsi_ctx *ctx) {
     // first: whatever else was recorded may come from what the wait was to bring
     if (h.tc_err != 0)
       return fail(ctx, QSI_ERR_TIMEOUT, "%s: bounded wait ran out (stage %d)",
-                  h.tc_err == QSI_STAGE_GJ32 ? "FP32 Gauss-Jordan" : "tensor-core kernel", h.tc_err);
+                  h.tc_err == QSI_STAGE_GJ32        ? "FP32 Gauss-Jordan"
+                  : h.tc_err == QSI_STAGE_INV_SMALL ? "FP64 inversion"
+                                                    : "tensor-core kernel",
+                  h.tc_err);
     if (h.code == QSI_ERR_SINGULAR)
       return fail(ctx, QSI_ERR_SINGULAR, "singular pivot: block %d (tip if %s), column %d", h.tag, "tag == n_blocks",
                   h.info);

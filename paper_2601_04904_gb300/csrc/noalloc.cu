@@ -37,10 +37,11 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void *g_addr[kMaxDevices] = {nullptr};
 
-// The singular-pivot report for the caller: 0, or 1 + the first bad column.
+// The report for the caller: 0, 1 + the first bad pivot column, or -1 after a
+// bounded wait that ran out.
 __global__ void noalloc_info_kernel(int32_t *info) {
   const QsiDevStatus *st = reinterpret_cast<const QsiDevStatus *>(g_noalloc_scratch);
-  *info = (st->code == (int)QSI_ERR_SINGULAR) ? st->info + 1 : 0;
+  *info = st->tc_err != 0 ? -1 : (st->code == (int)QSI_ERR_SINGULAR) ? st->info + 1 : 0;
 }
 
 }  // namespace

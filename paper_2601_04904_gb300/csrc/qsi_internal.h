@@ -20,6 +20,7 @@ struct QsiDevStatus {
 };
 // stages 1..5: the tensor-core products
 constexpr int QSI_STAGE_GJ32 = 6;        // cluster form of the FP32 Gauss-Jordan
+constexpr int QSI_STAGE_INV_SMALL = 7;   // FP64 inversion of a small block
 
 // Limit of a wait inside the inversion kernels, 2 s; QSI_INV_WAIT_NS in the
 // environment sets another one (0: no wait waits, all count as run out), for tests.

@@ -64,3 +64,45 @@ def test_batched_inversion_without_waits(ctx, monkeypatch):
     with pytest.raises(qsi.QsiError) as e:
         ctx.synchronize()
     assert e.value.status == qsi.ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("b", [9, 32, 40, 64])
+def test_small_fp64_inversion_without_waits(ctx, monkeypatch, b):
+    """The cluster form of the IEEE FP64 inversion, one and two row halves: reported by
+    the sweeps, and by the allocation-free inversion as info = -1."""
+    import ctypes
+    import torch
+    from paper_2601_04904_gb300 import build, qsi
+
+    n, a = 2, 3
+    h, B = inputs.hamiltonian(n, b, a), inputs.lesser_rhs(n, b, a)
+    A = ctx.assemble(qsi.to_device(h), 0.3, 1e-3, 0.5)
+    Bd = qsi.to_device(B)
+    block = torch.from_numpy(np.ascontiguousarray(rgf.assemble_a(h, 0.3, 1e-3, 0.5)["diag"][0])).cuda()
+    out, info = torch.empty_like(block), torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    lib = ctypes.CDLL(build.LIB)
+
+    def inverse():
+        assert lib.qsi_block_inverse_noalloc(ctypes.c_void_p(block.data_ptr()), ctypes.c_void_p(out.data_ptr()), b,
+                                             None, ctypes.c_void_p(info.data_ptr())) == 0
+        torch.cuda.synchronize()
+        return int(info.item())
+
+    with monkeypatch.context() as m:
+        m.setenv("QSI_INV_WAIT_NS", "0")
+        f = ctx.factor(A, Bd, qsi.FP64)
+        ctx.selquad(f)
+        with pytest.raises(qsi.QsiError, match="FP64 inversion: bounded wait ran out") as e:
+            ctx.synchronize()
+        f.close()
+        assert e.value.status == qsi.ERR_TIMEOUT
+        assert inverse() == -1
+    assert inverse() == 0
+    assert np.abs(out.cpu().numpy() @ block.cpu().numpy() - np.eye(b)).max() < 1e-11
+    f = ctx.factor(A, Bd, qsi.FP64)
+    GR, GL = ctx.selquad(f)
+    ctx.synchronize()
+    f.close()
+    oR, oL = rgf.selquad(rgf.assemble_a(h, 0.3, 1e-3, 0.5), B)
+    assert max_block_rel_err(qsi.to_host(GR), oR) < 1e-10 and max_block_rel_err(qsi.to_host(GL), oL) < 1e-10
