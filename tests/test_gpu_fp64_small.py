@@ -108,3 +108,20 @@ def test_wide_batches_of_small_blocks_give_the_bits_of_narrow_ones(ctx, b, point
     for i in (0, 1):
         for key in qsi.KEYS:
             assert (torch.cat([narrow[0][i][key], narrow[1][i][key]]) == wide[i][key]).all(), key
+
+
+@pytest.mark.parametrize("b,first", [(64, 0), (64, 7), (64, 31), (33, 31), (16, 7)])
+def test_the_first_of_several_singular_columns_is_reported(ctx, b, first):
+    """Zero columns on both sides of a boundary between CTAs (and every column after
+    the first, whose pivots are no longer finite): always the first one."""
+    from paper_2601_04904_gb300 import qsi
+
+    rng = np.random.default_rng(first)
+    a = rng.standard_normal((b, b)) + 1j * rng.standard_normal((b, b)) + 4 * np.eye(b)
+    a[:, [first, first + 1]] = 0
+    m = _single(qsi, a[None])[0]
+    for _ in range(30):
+        f = ctx.factor(m, None, qsi.FP64)
+        with pytest.raises(qsi.QsiError, match=f"column {first}$"):
+            ctx.synchronize()
+        f.close()
