@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const __grid_constant__
     __syncthreads();
     unsigned key = 0;
     if (cs > 1) {
-      asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      tc::cluster_sync();
       if (tid < CV_R * cs) {
         unsigned a, v;
         asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const __grid_constant__
         if (v != 0u) atomicMax(&s_all[tid % CV_R], v);
       }
       // no CTA leaves (or reuses s_key) while another may still read it: waited for at the end
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      tc::cluster_arrive();
       __syncthreads();
       key = s_all[r];
     } else {
@@ -464,10 +464,7 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const __grid_constant__
     else
       convert_four<NM < 0 ? 0 : NM, NP>(x, e, job.tbits, T, job.nmod, out, qplane);
   }
-  if (NM >= 0 && cs > 1) {
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
+  if (NM >= 0 && cs > 1) tc::cluster_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -672,7 +669,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_mma_kernel(const __grid_constan
       ok = __all_sync(0xffffffffu, ok && !*abort_flag);
       // all epilogue warps take the same decision before any further barrier
       if (lane == 0) epi_ok[ew] = ok ? 1 : 0;
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS));
+      named_sync(1, 32 * EPI_WARPS);
       bool all_ok = true;
 #pragma unroll
       for (int w = 0; w < EPI_WARPS; ++w) all_ok = all_ok && epi_ok[w];
@@ -764,7 +761,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_mma_kernel(const __grid_constan
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&accfree[buf]);
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS));  // staging complete (epilogue warps only)
+      named_sync(1, 32 * EPI_WARPS);  // staging complete (epilogue warps only)
       {
         // 16 bytes per lane, four rows per warp instruction (whole 32-byte
         // sectors): rows of res are a multiple of 16 long, so the last 16
@@ -797,9 +794,10 @@ __global__ void __launch_bounds__(THREADS, 1) tc_mma_kernel(const __grid_constan
             }
           }
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS));  // staging may be overwritten
+      named_sync(1, 32 * EPI_WARPS);  // staging may be overwritten
     }
   }
+  __syncwarp();  // the producer's and the issuer's lane rejoin their warps
   fence_before();
   __syncthreads();
   if (warp == 1) {
