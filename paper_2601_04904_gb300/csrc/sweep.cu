@@ -62,15 +62,13 @@ struct Group {
   }
 };
 
-const QsiExec *g_ex = nullptr;  // set by the sweep entry points (one sweep at a time per thread)
-
-cudaError_t run(Group &G, int batch, cudaStream_t s, QsiProf *prof) {
+cudaError_t run(const QsiExec &ex, Group &G, int batch, cudaStream_t s) {
   if (G.g.nprob == 0) return cudaSuccess;
-  if (g_ex && qsi_is_tc(g_ex->precision))
-    return qsi_zgemm_tc(G.g, batch, s, prof, g_ex->pool, &g_ex->status->tc_err,
-                        qsi_tc_scheme(g_ex->precision, g_ex->mixed_moduli),
-                        s == g_ex->st ? g_ex->arena_st : g_ex->arena_sd, &g_ex->tc_knobs);
-  return qsi_zgemm_fp64(G.g, batch, s, prof);
+  if (qsi_is_tc(ex.precision))
+    return qsi_zgemm_tc(G.g, batch, s, ex.prof, ex.pool, &ex.status->tc_err,
+                        qsi_tc_scheme(ex.precision, ex.mixed_moduli), s == ex.st ? ex.arena_st : ex.arena_sd,
+                        &ex.tc_knobs);
+  return qsi_zgemm_fp64(G.g, batch, s, ex.prof);
 }
 
 #define TRY(expr)                       \
@@ -182,7 +180,7 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
   // problems is launched first
   auto room = [&](Group &G, int k, cudaStream_t s) -> cudaError_t {
     if (G.g.nprob + k <= QSI_MAX_PROB) return cudaSuccess;
-    cudaError_t e = run(G, batch, s, prof);
+    cudaError_t e = run(ex, G, batch, s);
     G = Group();
     return e;
   };
@@ -259,7 +257,7 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
         TRY(room(G, 1, st));
         Group::term(G.add(bi, bi, T[r], bi), S, bi, ZOP_N, F.q[r].SB.at(oD(i)), bi, ZOP_N, bi);
       }
-      TRY(run(G, batch, st, prof));
+      TRY(run(ex, G, batch, st));
     }
     // F3
     {
@@ -278,7 +276,7 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
         TRY(room(G, 1, st));
         Group::term(G.add(bi, bi, F.q[r].SB.at(oD(i)), bi), T[r], bi, ZOP_N, S, bi, ZOP_H, bi);
       }
-      TRY(run(G, batch, st, prof));
+      TRY(run(ex, G, batch, st));
     }
     if (!quad) continue;
     TRY(cudaEventRecord(ex.ev_f3, st));
@@ -292,7 +290,7 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
         if (nx) Group::term(G.add(bn, bi, Q[r], bi), Alo, bi, ZOP_N, SBi, bi, ZOP_N, bi);
         if (a) Group::term(G.add(a, bi, W[r], bi), Abi, bi, ZOP_N, SBi, bi, ZOP_N, bi);
       }
-      TRY(run(G, batch, sd, prof));
+      TRY(run(ex, G, batch, sd));
     }
     // F5 (side stream); anti-Hermitian B: B-hat_{t,i+1} = -B-hat_{i+1,t}^H is mirrored
     {
@@ -333,7 +331,7 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
           Group::term(p3, Bbi, bi, ZOP_N, Lt, bi, ZOP_H, bi, MONE);
         }
       }
-      TRY(run(G, batch, sd, prof));
+      TRY(run(ex, G, batch, sd));
       TRY(run_mirror(mj, nm, batch, sd, prof));
     }
     TRY(cudaEventRecord(ex.ev_f5, sd));
@@ -347,12 +345,12 @@ static cudaError_t forward_steps(const QsiExec &ex, SweepArrays &F, zc *tmp) {
         TRY(room(G1, 1, st));
         Group::term(G1.add(a, a, T2[r], a), F.Stt, a, ZOP_N, F.q[r].SBtt, a, ZOP_N, a);
       }
-      TRY(run(G1, batch, st, prof));
+      TRY(run(ex, G1, batch, st));
       for (int r = 0; r < nr; ++r) {
         TRY(room(G2, 1, st));
         Group::term(G2.add(a, a, F.q[r].SBtt, a), T2[r], a, ZOP_N, F.Stt, a, ZOP_H, a);
       }
-      TRY(run(G2, batch, st, prof));
+      TRY(run(ex, G2, batch, st));
     }
   }
   return cudaSuccess;
@@ -376,7 +374,6 @@ cudaError_t qsi_sweep_forward(const QsiExec &ex_in, SweepArrays &F, zc *ws) {
   // temporaries from the pool when the caller gave none: with the shadow's room
   QsiExec ex = ex_in;
   if (!ws) ex.shadow_room = true;
-  g_ex = &ex;
   zc *tmp = ws;
   if (!tmp)
     TRY(cudaMallocFromPoolAsync((void **)&tmp,
@@ -465,7 +462,7 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
   auto ll = [&](int r, int i) { return L[r].l.p ? L[r].l.at(oU(i)) : Ll_s[r]; };
   auto room = [&](Group &G, int k, cudaStream_t s) -> cudaError_t {
     if (G.g.nprob + k <= QSI_MAX_PROB) return cudaSuccess;
-    cudaError_t e = run(G, batch, s, prof);
+    cudaError_t e = run(ex, G, batch, s);
     G = Group();
     return e;
   };
@@ -480,7 +477,7 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
       TRY(room(G, 1, st));
       G.add(a, a, L[r].t, a, F.q[r].SBtt, a, ONE);
     }
-    TRY(run(G, batch, st, prof));
+    TRY(run(ex, G, batch, st));
   }
   if (ex.out_tip) TRY(cudaEventRecord(ex.out_tip, st));
   const int first = F.partial ? n - 2 : n - 1;
@@ -550,7 +547,7 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
         Group::term(p, Xtt, a, ZOP_N, Abi, bi, ZOP_N, a);
       }
       TRY(split ? b1_g(G, st) : b1_sq(G, st));
-      TRY(run(G, batch, st, prof));
+      TRY(run(ex, G, batch, st));
     }
     if (split) {
       // the SQ step needs this step's U, P, G and the SI outputs of step i+1
@@ -558,7 +555,7 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
       TRY(wait_event(ex, sq, ex.ev_f3));
       Group G;
       TRY(b1_sq(G, sq));
-      TRY(run(G, batch, sq, prof));
+      TRY(run(ex, G, batch, sq));
     }
     // B2
     auto b2_sq = [&](Group &G, cudaStream_t s) -> cudaError_t {
@@ -599,12 +596,12 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
         Group::term(p, U2, w, ZOP_N, Xtt, a, ZOP_N, a, MONE);
       }
       if (!split) TRY(b2_sq(G, st));
-      TRY(run(G, batch, st, prof));
+      TRY(run(ex, G, batch, st));
     }
     if (split) {
       Group G;
       TRY(b2_sq(G, sq));
-      TRY(run(G, batch, sq, prof));
+      TRY(run(ex, G, batch, sq));
     }
     // B3
     auto b3_sq = [&](Group &G, cudaStream_t s) -> cudaError_t {
@@ -644,12 +641,12 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
         if (a) Group::term(p, U2, w, ZOP_N, R.bt.at(oR(i)), bi, ZOP_N, a, MONE);
       }
       if (!split) TRY(b3_sq(G, st));
-      TRY(run(G, batch, st, prof));
+      TRY(run(ex, G, batch, st));
     }
     if (split) {
       Group G;
       TRY(b3_sq(G, sq));
-      TRY(run(G, batch, sq, prof));
+      TRY(run(ex, G, batch, sq));
     }
     if (ex.ah_b && nl > 0) {
       // Y_{R,i} = -Y_{i,R}^H: the lower block (kept only when it is an output;
@@ -686,7 +683,7 @@ static cudaError_t backward_steps(const QsiExec &ex, const SweepArrays &F, const
         if (nx) Group::term(p, lu(r, i), bn, ZOP_N, U1, w, ZOP_H, bn, MONE);
         if (a) Group::term(p, Lr.r.at(oR(i)), a, ZOP_N, U2, w, ZOP_H, a, MONE);
       }
-      TRY(run(G, batch, sq, prof));
+      TRY(run(ex, G, batch, sq));
     }
     if (split) {
       TRY(cudaEventRecord(sq_done[par], sq));
@@ -719,7 +716,6 @@ size_t qsi_backward_tmp_elems(int b, int a, int batch, int nrhs, bool two_uv) {
 
 cudaError_t qsi_sweep_backward(const QsiExec &ex, const SweepArrays &F, const BtaView &GR, const BtaView *GL,
                                zc *ws) {
-  g_ex = &ex;
   zc *tmp = ws;
   if (!tmp)
     TRY(cudaMallocFromPoolAsync((void **)&tmp,
