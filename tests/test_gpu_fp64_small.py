@@ -125,3 +125,37 @@ def test_the_first_of_several_singular_columns_is_reported(ctx, b, first):
         with pytest.raises(qsi.QsiError, match=f"column {first}$"):
             ctx.synchronize()
         f.close()
+
+
+@pytest.mark.parametrize("m,n,k", [(128, 304, 9), (144, 272, 9), (150, 259, 40)])
+def test_product_kernels_either_side_of_the_line(ctx, m, n, k):
+    """152 tiles of 16 x 16 (128 x 304) take the 4 x 4 tiles, 153 (144 x 272) and more
+    the 16 x 16 ones: every op against numpy, nothing written past a row's end, and the
+    rows of a product the bits they have in a larger one across the line."""
+    import torch
+
+    rng = np.random.default_rng(m + n + k)
+    cn = lambda *s: rng.standard_normal(s) + 1j * rng.standard_normal(s)
+
+    def product(A, B, C, opA, opB):
+        nan = complex(float("nan"), float("nan"))
+        full = [torch.full((x.shape[0], x.shape[1] + 3), nan, dtype=torch.complex128, device="cuda") for x in (A, B, C)]
+        for d, x in zip(full, (A, B, C)):
+            d[:, :x.shape[1]].copy_(torch.from_numpy(x))
+        torch.cuda.synchronize()
+        dA, dB, dC = (d[:, :x.shape[1]] for d, x in zip(full, (A, B, C)))
+        ctx.zgemm(dA, dB, dC, opA=opA, opB=opB, alpha=-1.0, beta=1.0)
+        ctx.synchronize()
+        assert torch.isnan(full[2][:, C.shape[1]:].real).all() and torch.isnan(full[2][:, C.shape[1]:].imag).all()
+        return dC.cpu().numpy()
+
+    for opA in (0, 1):
+        for opB in (0, 1):
+            A, B, C = cn(*((k, m) if opA else (m, k))), cn(*((n, k) if opB else (k, n))), cn(m, n)
+            got = product(A, B, C, opA, opB)
+            ref = C - (A.conj().T if opA else A) @ (B.conj().T if opB else B)
+            scale = np.linalg.norm(A) * np.linalg.norm(B) + np.linalg.norm(C)
+            assert np.linalg.norm(got - ref) < 1e-15 * (k + 4) * scale
+            more = cn(*((k, 64) if opA else (64, k)))
+            large = product(np.concatenate([A, more], axis=1 if opA else 0), B, np.concatenate([C, cn(64, n)]), opA, opB)
+            assert (large[:m] == got).all()

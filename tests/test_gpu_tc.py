@@ -563,3 +563,22 @@ def test_product_tile_edges(ctx, precision, m, n, k):
             got = dev.cpu().numpy()
             scale = np.linalg.norm(A) * np.linalg.norm(B) + np.linalg.norm(C)
             assert np.linalg.norm(got - ref) < tol * scale
+
+
+@pytest.mark.parametrize("precision", ["fp64_emu", "mixed", "split3"])
+@pytest.mark.parametrize("m,n", [(1, 1), (17, 15), (33, 47), (129, 127), (260, 31)])
+def test_products_write_nothing_past_a_row(ctx, precision, m, n):
+    """The columns between N and the leading dimension keep what they held."""
+    import torch
+    from paper_2601_04904_gb300 import qsi
+
+    k, nan = 20, complex(float("nan"), float("nan"))
+    g = torch.Generator(device="cuda").manual_seed(m + n)
+    A, B = (torch.view_as_complex(torch.randn(r, c, 2, dtype=torch.float64, device="cuda", generator=g))
+            for r, c in ((m, k), (k, n)))
+    full = torch.full((m, n + 3), nan, dtype=torch.complex128, device="cuda")
+    torch.cuda.synchronize()
+    ctx.zgemm(A, B, full[:, :n], alpha=-1.0, precision=qsi.PRECISIONS[precision])
+    ctx.synchronize()
+    assert torch.isfinite(full[:, :n].real).all() and torch.isfinite(full[:, :n].imag).all()
+    assert torch.isnan(full[:, n:].real).all() and torch.isnan(full[:, n:].imag).all()
