@@ -410,8 +410,7 @@ def measure_batched(points=256, steps=2, warmup=1, precision="fp64_emu"):
     stk, ms_k = ctx.stats(), t0e.elapsed_time(t1e)
     shares = {k: stk[v] / ms_k for k, v in (("zinv_panel", "panel_ms"), ("fp32_gauss_jordan", "panel32_ms"),
                                             ("zgemm_fp64", "gemm_ms"), ("tc_mma", "tc_ms"), ("tc_aux", "tc_aux_ms"),
-                                            ("tc_aux_exp", "tc_exp_ms"), ("tc_aux_conv", "tc_conv_ms"),
-                                            ("tc_aux_crt", "tc_crt_ms"))}
+                                            ("tc_aux_conv", "tc_conv_ms"), ("tc_aux_crt", "tc_crt_ms"))}
     shares["zinv_other"] = (stk["inv_ms"] - stk["panel_ms"] - stk["panel32_ms"]) / ms_k
     # per-point single solves of the first points (same GPU), FP64 and `precision`
     k_single = min(8, nE)
@@ -772,10 +771,10 @@ def measure_c3(steps=3, warmup=2):
 # the kernels the roofline may name, keyed (kernel, precision), from one capture
 # of the kernel as it is now (cold caches: ncu flushes them between passes);
 # absent = not captured since the kernel last changed.
-TRAFFIC_PER_LAUNCH = {("tc_mma_kernel", "fp64_emu"): 1.188e8}
+TRAFFIC_PER_LAUNCH = {("tc_mma_kernel", "fp64_emu"): 7.65e7}
 TRAFFIC_SOURCE = {("tc_mma_kernel", "fp64_emu"):
-                  "ncu dram__bytes_read.sum + dram__bytes_write.sum, average over the 121 tc_mma launches of one "
-                  "step of the same block sizes on 8 blocks (caches flushed; "
+                  "ncu dram__bytes_read.sum + dram__bytes_write.sum, average over the 145 tc_mma launches "
+                  "of one step of the same block sizes on 8 blocks (caches flushed; "
                   "profiles/tc_mma_kernel_dram_bta_n8_b512_a256_fp64emu.md)"}
 
 
@@ -1138,7 +1137,6 @@ def main():
         "kernel_shares": {k: v / ms_kstep for k, v in (("zinv_panel", st["panel_ms"]), ("fp32_gauss_jordan", st["panel32_ms"]),
                                                        ("zgemm_fp64", st["gemm_ms"]), ("tc_mma", st["tc_ms"]),
                                                        ("tc_aux", st["tc_aux_ms"]),
-                                                       ("tc_aux_exp", st["tc_exp_ms"]),
                                                        ("tc_aux_conv", st["tc_conv_ms"]),
                                                        ("tc_aux_crt", st["tc_crt_ms"]),
                                                        ("zinv_other",

@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const __grid_constant__
 // 3. tensor-core products per modulus -> int8 residues of the exact integer
 //    product.  One CTA: one 128 x 128 complex output tile, mpc moduli (chosen
 //    per launch so that the CTAs fill the SMs in as few waves as possible).
-//    Warp 0: TMA producer; warp 1: TMEM owner + MMA issuer; warps 2..5:
+//    Warp 0: TMA producer; warp 1: TMEM owner + MMA issuer; warps 2..9:
 //    epilogue (TMEM -> residues -> shared staging -> coalesced global stores).
 //    TMEM: two buffers x (Cr | Ci), 4 x 128 columns.
 // ---------------------------------------------------------------------------
